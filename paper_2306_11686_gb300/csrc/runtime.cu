@@ -327,20 +327,24 @@ static void server_main(gf_ctx *c, uint32_t tid, uint32_t nthr)
 }
 
 /* ------------------------------------------------------------------ init / finalize */
+/* the arrays that a launch clears: the reset kernel writes whole 16-byte words */
+static uint64_t words16(uint64_t bytes) { return (bytes + 15) / 16; }
+static cudaError_t malloc16(void **p, uint64_t bytes) { return cudaMalloc(p, words16(bytes) * 16); }
+
 static int inst_alloc(gf_ctx *c, Instance *in)
 {
     const gf_config &cf = c->cfg;
     GF_CK(cudaMalloc((void **)&in->d_state, sizeof(gf_state)));
     GF_CK(cudaMalloc(&in->d_partials, (size_t)c->nsm * GF_MAX_BLOCKS_PER_SM * 16));
-    GF_CK(cudaMalloc(&in->d_fmt, (size_t)cf.fmt_cache * 8));
+    GF_CK(malloc16(&in->d_fmt, (size_t)cf.fmt_cache * 8));
     GF_CK(cudaMalloc((void **)&in->d_argv, GF_ARGV_BYTES));
     /* heap metadata, sized for the largest quota (the whole pool); the heap
      * itself is the launch's quota inside the context's pool */
-    GF_CK(cudaMalloc(&in->d_meta, (size_t)std::max<uint64_t>(c->max_slabs, 1) * 16));
-    GF_CK(cudaMalloc(&in->d_heads, (size_t)GF_MAX_SM * GF_HEAP_NCLASS * GF_HEAP_LANES * 8));
-    GF_CK(cudaMalloc(&in->d_cur, (size_t)GF_MAX_SM * GF_HEAP_NCLASS * 4));
+    GF_CK(malloc16(&in->d_meta, (size_t)std::max<uint64_t>(c->max_slabs, 1) * 16));
+    GF_CK(malloc16(&in->d_heads, (size_t)GF_MAX_SM * GF_HEAP_NCLASS * GF_HEAP_LANES * 8));
+    GF_CK(malloc16(&in->d_cur, (size_t)GF_MAX_SM * GF_HEAP_NCLASS * 4));
     GF_CK(cudaMalloc(&in->d_ext, (size_t)GF_LARGE_EXT_MAX * 8));
-    GF_CK(cudaMalloc(&in->d_lsize, (size_t)std::max<uint64_t>(c->max_pages, 1) * 4));
+    GF_CK(malloc16(&in->d_lsize, (size_t)std::max<uint64_t>(c->max_pages, 1) * 4));
     GF_CK(cudaEventCreateWithFlags(&in->ev_done, cudaEventDisableTiming));
     if (cf.split_regions)
         GF_CK(cudaStreamCreateWithFlags(&in->region_stream, cudaStreamNonBlocking));
@@ -813,7 +817,7 @@ extern "C" GF_API int gf_launch_q(gf_ctx *c, gf_program prog, int argc, const ch
  * own launch, this took the host and the stream about 60 us a program. */
 struct ResetArgs {
     uint4 *zero[5];
-    uint32_t zero_n[5];            /* 16-byte words */
+    uint32_t zero_n[5];            /* 16-byte words, of arrays padded to them */
     const uint64_t *init;
     uint64_t *state, *ext;
     const uint64_t *argv_from;
@@ -873,9 +877,7 @@ static int inst_start(gf_ctx *c, Instance *in, cudaStream_t stream, uint32_t gri
     H.nslabs = in->nslabs;
     H.npages = in->npages;
     H.large_next = in->npages ? 1 : 0;
-    /* every array is an allocation of its own, so a last 16-byte word may reach past its size */
     static_assert(sizeof(gf_state) % 8 == 0, "copied in words");
-    auto words16 = [](uint64_t bytes) { return (uint32_t)((bytes + 15) / 16); };
     ResetArgs a;
     void *const zero[5] = {in->d_meta, in->d_heads, in->d_cur, in->d_lsize, in->d_fmt};
     const uint64_t bytes[5] = {(uint64_t)std::max<uint32_t>(in->nslabs, 1) * 16,
@@ -884,7 +886,7 @@ static int inst_start(gf_ctx *c, Instance *in, cudaStream_t stream, uint32_t gri
                                (uint64_t)c->cfg.fmt_cache * 8};
     for (int z = 0; z < 5; z++) {
         a.zero[z] = (uint4 *)zero[z];
-        a.zero_n[z] = words16(bytes[z]);
+        a.zero_n[z] = (uint32_t)words16(bytes[z]);
     }
     a.init = (const uint64_t *)in->pin_dev;
     a.state = (uint64_t *)in->d_state;

@@ -1,0 +1,203 @@
+/*
+ * Host-only test of a launch's device state: runtime.cu compiled against a
+ * fake CUDA runtime whose device memory is host memory of exactly the sizes
+ * asked for, and whose stream holds the reset kernel back until something
+ * waits for the stream.
+ *
+ *   launch_fake_cuda <scenario>
+ *
+ * Scenarios (each prints "OK" and exits 0, or prints the failure and exits 1):
+ *   reset    what the reset kernel is told to write lies inside the
+ *            allocations, over configurations whose arrays are small or odd
+ */
+#include <cuda_runtime.h>
+#include <cstdint>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+#include <vector>
+
+namespace fake {
+std::map<uint64_t, uint64_t> mem;                 /* allocations: address, bytes asked for */
+struct Kernel {
+    cudaStream_t stream;
+    std::vector<char> args;
+};
+std::vector<Kernel> queued;                       /* reset kernels that have not run */
+std::string trouble;
+size_t arg_bytes = 0;
+void run(const std::vector<char> &args);          /* the reset kernel on the host */
+
+template <class T> cudaError_t alloc(T **p, size_t n)
+{
+    *p = (T *)calloc(1, n + 64);
+    mem[(uint64_t)*p] = n;
+    return cudaSuccess;
+}
+cudaError_t release(void *p)
+{
+    mem.erase((uint64_t)p);
+    free(p);
+    return cudaSuccess;
+}
+bool inside(uint64_t a, uint64_t n)
+{
+    auto it = mem.upper_bound(a);
+    return n == 0 || (it != mem.begin() && (--it, a + n <= it->first + it->second));
+}
+template <class T> cudaError_t make(T *p)
+{
+    *p = (T)malloc(1);
+    return cudaSuccess;
+}
+cudaError_t drop(void *p)
+{
+    free(p);
+    return cudaSuccess;
+}
+cudaError_t drain(cudaStream_t s)
+{
+    for (size_t k = 0; k < queued.size();)
+        if (queued[k].stream == s) {
+            run(queued[k].args);
+            queued.erase(queued.begin() + (long)k);
+        } else {
+            k++;
+        }
+    return cudaSuccess;
+}
+cudaError_t launch(void **args, cudaStream_t s)
+{
+    const char *a = (const char *)args[0];
+    queued.push_back({s, std::vector<char>(a, a + arg_bytes)});
+    return cudaSuccess;
+}
+int copies_fail = 0;                              /* the next asynchronous copies fail */
+cudaError_t copy(void *d, const void *s, size_t n, cudaStream_t st)
+{
+    if (copies_fail) {
+        copies_fail--;
+        return cudaErrorUnknown;
+    }
+    drain(st);
+    memcpy(d, s, n);
+    return cudaSuccess;
+}
+template <class T> cudaError_t is(T *p, T v)
+{
+    *p = v;
+    return cudaSuccess;
+}
+cudaError_t dev_pointer(cudaPointerAttributes *a)
+{
+    memset(a, 0, sizeof *a);
+    a->type = cudaMemoryTypeDevice;
+    return cudaSuccess;
+}
+} // namespace fake
+
+#define cudaMalloc(p, n) fake::alloc(p, n)
+#define cudaMallocAsync(p, n, s) fake::alloc(p, n)
+#define cudaHostAlloc(p, n, f) fake::alloc(p, n)
+#define cudaFree(p) fake::release(p)
+#define cudaFreeAsync(p, s) fake::release(p)
+#define cudaFreeHost(p) fake::release(p)
+#define cudaHostGetDevicePointer(d, h, f) fake::is((void **)(d), (void *)(h))
+#define cudaPointerGetAttributes(a, p) fake::dev_pointer(a)
+#define cudaStreamCreateWithFlags(s, f) fake::make(s)
+#define cudaEventCreateWithFlags(e, f) fake::make(e)
+#define cudaStreamDestroy(s) fake::drop(s)
+#define cudaEventDestroy(e) fake::drop(e)
+#define cudaEventRecord(e, s) cudaSuccess
+#define cudaEventQuery(e) cudaSuccess
+#define cudaEventSynchronize(e) cudaSuccess
+#define cudaStreamSynchronize(s) fake::drain(s)
+#define cudaMemcpyAsync(d, s, n, k, st) fake::copy((void *)(d), (const void *)(s), n, st)
+#define cudaLaunchKernel(f, g, b, args, shm, s) fake::launch(args, s)
+#define cudaSetDevice(d) cudaSuccess
+#define cudaGetDevice(d) fake::is(d, 0)
+#define cudaDeviceGetAttribute(v, a, d) fake::is(v, 152)
+#define cudaDeviceGetLimit(v, l) fake::is(v, (size_t)4096)
+#define cudaDeviceSetLimit(l, v) cudaSuccess
+
+#include "runtime.cu"
+
+void fake::run(const std::vector<char> &args)
+{
+    ResetArgs a;
+    memcpy((void *)&a, args.data(), sizeof a);
+    auto span = [&](const char *what, const void *p, uint64_t n) {
+        if (!inside((uint64_t)p, n))
+            trouble += std::string(what) + " reaches past its allocation\n";
+    };
+    span("state", a.state, a.init_n * 8ull);
+    span("initial state", a.init, a.init_n * 8ull);
+    span("argv", a.argv_to, a.argv_n * 8ull);
+    span("argv source", a.argv_from, a.argv_n * 8ull);
+    span("extents", a.ext, 8);
+    for (int z = 0; z < 5; z++)
+        span(("array " + std::to_string(z)).c_str(), a.zero[z], a.zero_n[z] * 16ull);
+    if (!trouble.empty())
+        return;
+    memcpy(a.state, a.init, a.init_n * 8ull);
+    memcpy(a.argv_to, a.argv_from, a.argv_n * 8ull);
+    a.ext[0] = a.ext0;
+    for (int z = 0; z < 5; z++)
+        memset(a.zero[z], 0, a.zero_n[z] * 16ull);
+}
+
+static cudaError_t prog_launch(void **, unsigned, unsigned, void *) { return cudaSuccess; }
+static int prog_occ(unsigned) { return 2; }
+
+static int prog()
+{
+    return gf_program_register("fake", prog_launch, prog_occ, prog_launch);
+}
+
+static gf_config config()
+{
+    gf_config c;
+    gf_config_default(&c);
+    c.heap_bytes = 1 << 20;
+    c.ring_slots = 8;
+    c.server_threads = 0;
+    c.bulk_bytes = 0;
+    return c;
+}
+
+static bool reset()
+{
+    const int p = prog();
+    const char *argv[2] = {"fake", "x"};
+    for (uint64_t heap : {0ull, 1ull, 256ull << 10, 1ull << 20, (3ull << 20) + 1})
+        for (uint32_t pct : {0u, 50u, 100u})
+            for (uint32_t fmt : {1u, 2u, 4096u})
+                for (int argc : {0, 1, 2}) {
+                    gf_config cf = config();
+                    cf.heap_bytes = heap;
+                    cf.heap_small_pct = pct;
+                    cf.fmt_cache = fmt;
+                    gf_ctx *c = nullptr;
+                    gf_handle *h = nullptr;
+                    int ec = 0;
+                    if (gf_init(&cf, &c) || gf_launch(c, p, argc, argv, nullptr, 0, nullptr, 0, &h) || gf_wait(h, &ec, 0))
+                        fake::trouble += "a launch failed\n";
+                    gf_finalize(c);
+                    if (!fake::trouble.empty()) {
+                        printf("heap %llu pct %u fmt_cache %u argc %d\n", (unsigned long long)heap, pct, fmt, argc);
+                        return false;
+                    }
+                }
+    return true;
+}
+
+int main(int argc, char **argv)
+{
+    fake::arg_bytes = sizeof(ResetArgs);
+    const std::string s = argc > 1 ? argv[1] : "";
+    const bool ok = s == "reset" && reset();
+    printf("%s%s\n", fake::trouble.c_str(), ok && fake::trouble.empty() ? "OK" : "FAILED");
+    return ok && fake::trouble.empty() ? 0 : 1;
+}
