@@ -759,6 +759,8 @@ extern "C" GF_API int gf_launch_q(gf_ctx *c, gf_program prog, int argc, const ch
     in->region = pe.region;
     in->region_grid = region_grid;
     auto bail = [&](int e) {
+        /* what is queued (the reset kernel reads the instance's mapped block) ends before the instance goes */
+        cudaStreamSynchronize(h->stream);
         release_staged(h, false);
         seg_stop(c, in);
         inst_release(c, in);
@@ -942,9 +944,9 @@ int gf_inst_finish(gf_ctx *c, int idx, void *stream)
 {
     Instance *in = c->inst[(size_t)idx];
     in->h_final()->rpc_ticket = ~0ull;
-    if (cudaMemcpyAsync(in->h_final(), in->d_state, sizeof(gf_state), cudaMemcpyDeviceToHost, (cudaStream_t)stream) !=
-            cudaSuccess ||
-        cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess)
+    const cudaError_t copied =
+        cudaMemcpyAsync(in->h_final(), in->d_state, sizeof(gf_state), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
+    if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess || copied != cudaSuccess)
         return GF_ECUDA;
     in->borrowed_tickets = in->h_final()->rpc_ticket;
     return in->h_final()->error;
@@ -1013,6 +1015,7 @@ extern "C" GF_API int gf_wait(gf_handle *h, int *exit_code, int64_t timeout_ns)
         if (q != cudaErrorNotReady) {
             fprintf(stderr, "gf: program failed: %s\n", cudaGetErrorString(q));
             seg_stop(c, in);
+            cudaStreamSynchronize(h->stream);
             release_staged(h, false);
             ring_used(c, in, ~0ull);
             inst_release(c, in);

@@ -9,6 +9,8 @@
  * Scenarios (each prints "OK" and exits 0, or prints the failure and exits 1):
  *   reset    what the reset kernel is told to write lies inside the
  *            allocations, over configurations whose arrays are small or odd
+ *   failed   a launch or a borrow that fails after the reset kernel was queued
+ *            gives the instance back only when that kernel has run
  */
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -149,6 +151,7 @@ void fake::run(const std::vector<char> &args)
 }
 
 static cudaError_t prog_launch(void **, unsigned, unsigned, void *) { return cudaSuccess; }
+static cudaError_t prog_refused(void **, unsigned, unsigned, void *) { return cudaErrorUnknown; }
 static int prog_occ(unsigned) { return 2; }
 
 static int prog()
@@ -193,11 +196,41 @@ static bool reset()
     return true;
 }
 
+static bool failed()
+{
+    const int good = prog(), bad = gf_program_register("refused", prog_refused, prog_occ, prog_launch);
+    const gf_config cf = config();
+    gf_ctx *c = nullptr;
+    gf_handle *h = nullptr;
+    int ec = 0, idx = -1, other = 0;
+    if (gf_init(&cf, &c))
+        return false;
+    if (gf_launch(c, bad, 0, nullptr, nullptr, 0, &other, 0, &h) != GF_ECUDA || h)
+        fake::trouble += "the refused launch did not fail\n";
+    if (!fake::queued.empty())
+        fake::trouble += "a failed launch leaves its reset kernel behind\n";
+    fake::drain((cudaStream_t)&other);
+    if (!gf_inst_acquire(c, &other, 1, &idx))
+        return false;
+    fake::copies_fail = 1;
+    if (gf_inst_finish(c, idx, &other) != GF_ECUDA)
+        fake::trouble += "the failed copy is not reported\n";
+    if (!fake::queued.empty())
+        fake::trouble += "a failed copy leaves the reset kernel behind\n";
+    gf_inst_release(c, idx);
+    fake::drain((cudaStream_t)&other);
+    /* and the instance serves the next program */
+    if (gf_launch(c, good, 0, nullptr, nullptr, 0, nullptr, 0, &h) || gf_wait(h, &ec, 0))
+        fake::trouble += "the next launch failed\n";
+    gf_finalize(c);
+    return true;
+}
+
 int main(int argc, char **argv)
 {
     fake::arg_bytes = sizeof(ResetArgs);
     const std::string s = argc > 1 ? argv[1] : "";
-    const bool ok = s == "reset" && reset();
+    const bool ok = s == "reset" ? reset() : s == "failed" && failed();
     printf("%s%s\n", fake::trouble.c_str(), ok && fake::trouble.empty() ? "OK" : "FAILED");
     return ok && fake::trouble.empty() ? 0 : 1;
 }

@@ -1,5 +1,6 @@
 """A launch's host side with a fake CUDA runtime (no GPU): what the reset
-kernel writes lies inside the instance's allocations."""
+kernel writes lies inside the instance's allocations, and an instance goes to
+the next program only when that kernel has run, also where a launch fails."""
 import os
 import subprocess
 
@@ -18,7 +19,7 @@ def launch_bin(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["reset"])
+@pytest.mark.parametrize("scenario", ["reset", "failed"])
 def test_launch_scenario(launch_bin, scenario):
     p = subprocess.run([launch_bin, scenario], capture_output=True, text=True, timeout=120)
     assert p.returncode == 0, p.stdout + p.stderr
