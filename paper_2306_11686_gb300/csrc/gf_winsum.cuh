@@ -8,8 +8,9 @@
  * has p = e - base in [0, 31] is the 53-bit significand shifted left by p,
  * added (its one's complement for a negative value, whose missing +1s are
  * counted) to a 96-bit integer in units of 2^(base - 1075): about 16 integer
- * instructions, no rounding.  With 53 + 31 bits a term, 2^11 terms fit; the
- * accumulator is then folded into a double pair.  (Fixed-point accumulation in
+ * instructions, no rounding.  With 53 + 31 bits a term, 2^11 terms fit: the
+ * one that opens a window and GF_WIN_TERMS more, after which the accumulator
+ * is folded into a double pair.  (Fixed-point accumulation in
  * the manner of U. Kulisch, "Computer Arithmetic and Validity", with a short
  * register that moves.)
  *
@@ -24,7 +25,7 @@
 #define GF_WINSUM_CUH
 #include "gf_intpipe.cuh"
 
-#define GF_WIN_TERMS 2048u       /* terms between two folds */
+#define GF_WIN_TERMS 2047u       /* terms between two folds, besides one that add_out adds */
 #define GF_WIN_TOP 1900u         /* highest exponent that makes a window */
 
 struct gf_winsum {
