@@ -134,6 +134,10 @@ GF_IP_HD uint64_t gf_fs_third(uint32_t lo, uint32_t hi)
     return (uint64_t)hi * 0x55555555u + (uint32_t)(w2 >> 32);
 }
 
+/* The highest window's top: its values lie below 2^(2044 - 1023) = 2^1021, so six of them sum below 2^1024.  One
+ * binade higher the FP64 sum can overflow to infinity, and the chunks' sum does not. */
+#define GF_FIX_TOP 2043u
+
 struct gf_fix3 {
     float a, b, c;
 };

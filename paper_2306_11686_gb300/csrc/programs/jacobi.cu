@@ -451,7 +451,7 @@ static __device__ uint32_t jacobi_window(const double *u, uint32_t cells, int *r
     jacobi_red red{0ull, 0, 0u};
     *rc = jacobi_sample(u, cells, 0u, &red);
     const uint32_t top = (uint32_t)red.hi >> 20;
-    if (*rc || top < 13u || top > 2044u)
+    if (*rc || top < 13u || top > GF_FIX_TOP)
         return 0u;
     *rc = jacobi_sample(u, cells, top - 8u, &red);
     return *rc || red.out > JACOBI_SAMPLE / 4096 ? 0u : top - 8u;
@@ -540,7 +540,7 @@ GF_MAIN_HOT(jacobi, 2, jacobi_hot)(int argc, char **argv)
                 rc = jacobi_rest(u, un, nn, (uint32_t)cells, &rest);
             res = __longlong_as_double((long long)max(red.res, rest.res));
             const uint32_t top = (uint32_t)max(red.hi, rest.hi) >> 20;
-            elow = top < 13u || top > 2044u || red.out > cells / 64 ? 0u : top - 8u;
+            elow = top < 13u || top > GF_FIX_TOP || red.out > cells / 64 ? 0u : top - 8u;
             ask = 0;
         } else if (argc <= 4) {
             rc = jacobi_sweep<0>(u, un, nn, dn, cells, &res);
