@@ -183,7 +183,8 @@ typedef struct gf_state {
     gf_region region;
     uint64_t red_result[2];
     /* configuration written by the host before launch */
-    uint32_t nblocks, block_dim, nworkers, aggregate;
+    uint32_t nblocks, block_dim;  /* the program kernel's                                */
+    uint32_t nworkers, aggregate; /* threads that run a region (kernel split: the region kernel's) */
     int64_t timeout_ns;
     uint64_t ring_slots;       /* device address of the mapped slot array            */
     uint32_t nslots, slot_bytes;

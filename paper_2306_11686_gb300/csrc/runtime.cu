@@ -851,7 +851,7 @@ static int inst_start(gf_ctx *c, Instance *in, cudaStream_t stream, uint32_t gri
     gf_state &s = *in->h_init();
     s.nblocks = grid;
     s.block_dim = GF_BLOCK_THREADS;
-    s.nworkers = grid * GF_BLOCK_THREADS - 32;
+    s.nworkers = c->cfg.split_regions ? in->region_grid * GF_BLOCK_THREADS : grid * GF_BLOCK_THREADS - 32;
     s.aggregate = c->cfg.aggregate;
     s.timeout_ns = c->cfg.timeout_ns;
     s.ring_slots = c->ring_dev + in->ring_first * c->cfg.slot_bytes;

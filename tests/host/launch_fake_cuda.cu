@@ -11,6 +11,8 @@
  *            allocations, over configurations whose arrays are small or odd
  *   failed   a launch or a borrow that fails after the reset kernel was queued
  *            gives the instance back only when that kernel has run
+ *   split    the state of a program whose regions are kernels of their own
+ *            counts the threads of the region kernel as workers
  */
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -226,11 +228,38 @@ static bool failed()
     return true;
 }
 
+static bool split()
+{
+    const int p = prog();
+    for (uint32_t grid : {0u, 1u, 5u, 304u})
+        for (uint32_t mode : {0u, 1u}) {
+            gf_config cf = config();
+            cf.split_regions = mode;
+            cf.server_threads = 1;
+            gf_ctx *c = nullptr;
+            gf_handle *h = nullptr;
+            int ec = 0;
+            if (gf_init(&cf, &c) || gf_launch(c, p, 0, nullptr, nullptr, 0, nullptr, grid, &h))
+                return false;
+            const uint32_t all = grid ? grid : 304u;                       /* two blocks on each of 152 SMs */
+            const uint32_t want = mode ? 256u * (all == 304u ? 303u : all) : 256u * all - 32u;
+            const uint32_t got = h->inst->h_init()->nworkers;
+            if (got != want) {
+                printf("grid %u split %u: %u workers, not %u\n", grid, mode, got, want);
+                return false;
+            }
+            if (gf_wait(h, &ec, 0))
+                return false;
+            gf_finalize(c);
+        }
+    return true;
+}
+
 int main(int argc, char **argv)
 {
     fake::arg_bytes = sizeof(ResetArgs);
     const std::string s = argc > 1 ? argv[1] : "";
-    const bool ok = s == "reset" ? reset() : s == "failed" && failed();
+    const bool ok = s == "reset" ? reset() : s == "failed" ? failed() : s == "split" && split();
     printf("%s%s\n", fake::trouble.c_str(), ok && fake::trouble.empty() ? "OK" : "FAILED");
     return ok && fake::trouble.empty() ? 0 : 1;
 }
