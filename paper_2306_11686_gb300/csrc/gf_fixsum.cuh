@@ -113,7 +113,7 @@ GF_IP_HD uint32_t gf_fs_shr(uint32_t lo, uint32_t hi, uint32_t k)
     return (uint32_t)((((uint64_t)hi << 32) | lo) >> k);
 #endif
 }
-/* leading zeros of x != 0 */
+/* leading zeros of x; 2^32 - 1 for x = 0 */
 GF_IP_HD uint32_t gf_fs_clz(uint32_t x)
 {
 #ifdef __CUDA_ARCH__
@@ -121,7 +121,7 @@ GF_IP_HD uint32_t gf_fs_clz(uint32_t x)
     asm("bfind.shiftamt.u32 %0, %1;" : "=r"(r) : "r"(x));
     return r;
 #else
-    return (uint32_t)__builtin_clz(x | !x);
+    return x ? (uint32_t)__builtin_clz(x) : 0xffffffffu;
 #endif
 }
 
@@ -178,16 +178,17 @@ GF_IP_HD gf_fix3 gf_fix_add(gf_fix3 x, gf_fix3 y)
     return r;
 }
 
-/* the sum is a positive number of the window's units: neither 0 nor NaN */
-GF_IP_HD bool gf_fix_ok(gf_fix3 t) { return t.a > 0.0f; }
+/* the sum is a number of the window's units, not NaN (0 where all its values are +0) */
+GF_IP_HD bool gf_fix_ok(gf_fix3 t) { return t.a >= 0.0f; }
 
 /* RN(t / 6) for a sum t of at most six values with gf_fix_ok, each add rounded */
 GF_IP_HD double gf_fix_div6(gf_fix3 t, uint32_t elow)
 {
-    /* T in units, 2^52 <= T < 6 * 2^61 < 2^64 */
+    /* T in units, 0 or 2^52 <= T < 6 * 2^61 < 2^64 */
     const uint64_t bc = (uint64_t)(uint32_t)(t.b * 1.9073486328125e-06f) * 524288u + (uint32_t)t.c;
     const uint32_t th = (uint32_t)(bc >> 32) + (uint32_t)(t.a * 2.3283064365386963e-10f), tl = (uint32_t)bc;
-    const uint32_t z = gf_fs_clz(th);
+    /* at most 11; T = 0 takes the z that makes the result's exponent field 0 (elow >= 5), and all shifts leave 0 */
+    const uint32_t zt = gf_fs_clz(th), z = zt < elow + 7u ? zt : elow + 7u;
     const uint32_t nh = gf_fs_shl(tl, th, z), nl = gf_fs_shl1(tl, z);          /* leading bit at 63, 11 zero bits below */
     const uint32_t s = nh < 0xc0000000u ? 9u : 10u;                  /* n = T 2^z >> s: n / 3 in [2^52, 2^53) */
     const uint32_t qh = nh >> s, ql = gf_fs_shr(nl, nh, s);

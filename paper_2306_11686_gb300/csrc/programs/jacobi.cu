@@ -358,7 +358,7 @@ struct jacobi_fix_body {
                     }
                 }
                 uint32_t bh[R], bl[R], big = 0u;       /* the residuals' bits */
-                float least = 1.0f;                    /* NaN or 0: a sum was not computed here */
+                float least = 1.0f;                    /* NaN: a sum was not computed here */
 #pragma unroll
                 for (int q = 0; q < R; q++) {
                     m[q] = c[q];
@@ -373,7 +373,7 @@ struct jacobi_fix_body {
                     big = max(big, bh[q]);
                     asm("min.NaN.f32 %0, %0, %1;" : "+f"(least) : "f"(s[q].a));
                 }
-                if (__any_sync(0xffffffffu, in != 0u && (big >= top || !(least > 0.0f)))) {
+                if (__any_sync(0xffffffffu, in != 0u && (big >= top || !(least >= 0.0f)))) {
                     big = top;
                     const uint32_t before = left;
 #pragma unroll
@@ -445,12 +445,15 @@ static __device__ int jacobi_sample(const double *u, uint32_t cells, uint32_t el
 }
 
 /* the lowest binade (biased exponent) of the fixed-point window that suits the grid u, 0 if none does: less
- * than one value in 4096 may lie outside it (each costs up to six points the FP64 path) */
+ * than one value in 4096 may lie outside it (each costs up to six points the FP64 path).  +0 lies in every
+ * window; a sample of nothing else takes the one that ends at 2, and the first sweep sees what there is. */
 static __device__ uint32_t jacobi_window(const double *u, uint32_t cells, int *rc)
 {
     jacobi_red red{0ull, 0, 0u};
     *rc = jacobi_sample(u, cells, 0u, &red);
     const uint32_t top = (uint32_t)red.hi >> 20;
+    if (!*rc && red.hi == 0 && red.out == 0u)
+        return 1015u;
     if (*rc || top < 13u || top > GF_FIX_TOP)
         return 0u;
     *rc = jacobi_sample(u, cells, top - 8u, &red);
@@ -539,8 +542,11 @@ GF_MAIN_HOT(jacobi, 2, jacobi_hot)(int argc, char **argv)
             if (!rc && red.out)
                 rc = jacobi_rest(u, un, nn, (uint32_t)cells, &rest);
             res = __longlong_as_double((long long)max(red.res, rest.res));
-            const uint32_t top = (uint32_t)max(red.hi, rest.hi) >> 20;
-            elow = top < 13u || top > GF_FIX_TOP || red.out > cells / 64 ? 0u : top - 8u;
+            const uint32_t hi = (uint32_t)max(red.hi, rest.hi), top = hi >> 20;
+            if (red.out > cells / 64)
+                elow = 0u;
+            else if (hi != 0u)                     /* 0: nothing but zeros was seen */
+                elow = top < 13u || top > GF_FIX_TOP ? 0u : top - 8u;
             ask = 0;
         } else if (argc <= 4) {
             rc = jacobi_sweep<0>(u, un, nn, dn, cells, &res);
