@@ -543,11 +543,14 @@ GF_MAIN_HOT(jacobi, 2, jacobi_hot)(int argc, char **argv)
                 rc = jacobi_rest(u, un, nn, (uint32_t)cells, &rest);
             res = __longlong_as_double((long long)max(red.res, rest.res));
             const uint32_t hi = (uint32_t)max(red.hi, rest.hi), top = hi >> 20;
-            if (red.out > cells / 64)
+            if (red.out > cells / 64) {            /* the window does not suit: the FP64 pipe for a while */
                 elow = 0u;
-            else if (hi != 0u)                     /* 0: nothing but zeros was seen */
-                elow = top < 13u || top > GF_FIX_TOP ? 0u : top - 8u;
-            ask = 0;
+                ask = pause;
+            } else {
+                if (hi != 0u)                      /* 0: nothing but zeros was seen */
+                    elow = top < 13u || top > GF_FIX_TOP ? 0u : top - 8u;
+                ask = pause = 0;
+            }
         } else if (argc <= 4) {
             rc = jacobi_sweep<0>(u, un, nn, dn, cells, &res);
         } else if (kseg > 0) {
