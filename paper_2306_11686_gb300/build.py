@@ -23,7 +23,7 @@ NVFLAGS = ARCH + INC + ["-O3", "-lineinfo", "-std=c++17", "--fmad=false", "-Xcom
                         "-Xptxas", "-v", "-diag-suppress", "177"]
 CXXFLAGS = INC + ["-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-Wall"]
 
-CU = ["runtime.cu", "noalloc.cu", "peak.cu", "programs/legacy.cu", "programs/jacobi.cu",
+CU = ["runtime.cu", "noalloc.cu", "peak.cu", "programs/legacy.cu", "programs/jacobi.cu", "programs/jacobi_fp64.cu",
       "programs/probes_sched.cu", "programs/probes_rpc.cu",
       "programs/probes_heap.cu", "programs/probes_misc.cu", "programs/stress.cu", "programs/batch.cu",
       "programs/synth.cu", "programs/serve.cu",
@@ -31,7 +31,7 @@ CU = ["runtime.cu", "noalloc.cu", "peak.cu", "programs/legacy.cu", "programs/jac
 CPP = ["host/server.cpp", "host/mlp.cpp"]
 HEADERS = ["gf_layout.h", "gf_device.cuh", "gf_device_rpc.cuh", "gf_device_heap.cuh", "gf_program.h",
            "host/server.h", "host/range_alloc.h", "gf_errors.h", "gf_internal.h", "gf_fastdiv.cuh", "gf_paper_alloc.cuh", "gf_device_libc.cuh",
-           "gf_intpipe.cuh", "gf_fixsum.cuh", "gf_winsum.cuh", "gf_strtod_fast.h", "host/fmt_fast.h", "host/dtoa_fixed.h"]
+           "gf_intpipe.cuh", "gf_fixsum.cuh", "gf_winsum.cuh", "programs/jacobi.cuh", "gf_strtod_fast.h", "host/fmt_fast.h", "host/dtoa_fixed.h"]
 
 
 def _newer(obj, deps):

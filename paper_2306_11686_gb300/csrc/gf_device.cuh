@@ -719,11 +719,11 @@ template <class T, int OP, class F> struct hot_reduce {
     }
 };
 
-template <class HOT> static __device__ __noinline__ void worker_loop(gf_state *S)
+template <class HOT> static __device__ __noinline__ void worker_loop(gf_state *S, uint32_t epoch0)
 {
     const wctx w = make_wctx();
     const bool first = threadIdx.x >> 5 == w.wfirst;     /* the poller's warp */
-    uint32_t seen = 0;
+    uint32_t seen = epoch0;
     /* idle bound: the serial part may run long, but not forever */
     const uint64_t idle_limit = 8ull * (uint64_t)S->timeout_ns;
     for (;;) {
@@ -1018,29 +1018,64 @@ namespace gfd {
 typedef int (*main_t)(int, char **);
 
 /* MINB: resident blocks per SM the kernel is compiled for (a register cap);
- * memory-bound programs ask for more resident warps with GF_MAIN_BOUNDS. */
-template <main_t MAIN, int MINB = GF_MIN_BLOCKS, class HOT = no_hot>
+ * memory-bound programs ask for more resident warps with GF_MAIN_BOUNDS.
+ * SECOND: the program's second kernel (GF_SECOND).  It runs main when the
+ * launch took it alone or the first kernel's main called gf_second_kernel; in
+ * the latter case epoch and done_blocks go on from the first kernel's, whose
+ * blocks have all left. */
+template <main_t MAIN, int MINB = GF_MIN_BLOCKS, class HOT = no_hot, bool SECOND = false>
 __global__ void __launch_bounds__(GF_BLOCK, MINB) program_kernel(gf_state *S, int argc, char **argv)
 {
+    if (SECOND && *(volatile uint32_t *)&S->second == 0u)
+        return;
     if (threadIdx.x == 0)
         block_setup(S, 0);
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x < 32) {
         if (threadIdx.x == 0) {
-            S->t_main_start = now_ns();
+            if (SECOND) {
+                s_main_epoch = S->epoch0;
+                s_done_target = S->done0;
+                S->nblocks = gridDim.x;
+                S->nworkers = S->split ? S->nworkers : gridDim.x * GF_BLOCK - 32;
+            }
+            if (!SECOND || S->second == 1u)
+                S->t_main_start = now_ns();
             int rc = MAIN(argc, argv);
             pb_flush(S);                      /* printf records main left buffered */
             rpc_collect_deferred(S, false);   /* a printf main did not wait for */
             S->exit_code = rc;
             S->t_main_end = now_ns();
+            if (!SECOND) {
+                S->epoch0 = s_main_epoch + 1u;
+                S->done0 = s_done_target;
+            }
             S->main_done = 1;
             S->region.fn = 0;                 /* the workers leave their loop */
             st_rel_gpu(&S->epoch, ++s_main_epoch);
         }
         return;
     }
-    worker_loop<HOT>(S);
+    worker_loop<HOT>(S, SECOND ? S->epoch0 : 0u);
 }
+
+} // namespace gfd
+
+/* From the first kernel's main, which then returns: the rest of the program
+ * runs on its second kernel, whose main finds the two words in
+ * gf_state::second_arg.  False where no second kernel is queued. */
+__device__ __forceinline__ bool gf_second_kernel(uint64_t a, uint64_t b)
+{
+    gf_state *S = gfd::s_st;
+    if (!S->second_follows)
+        return false;
+    S->second_arg[0] = a;
+    S->second_arg[1] = b;
+    S->second = 2u;
+    return true;
+}
+
+namespace gfd {
 
 /*
  * The kernel split's region kernel (paper Sec. 3.3, Fig. 3), a comparator:
@@ -1073,18 +1108,18 @@ __global__ void __launch_bounds__(GF_BLOCK, MINB) region_kernel(gf_state *S)
 /* host-side registration of a program (name -> cooperative launcher) */
 #include "gf_program.h"
 
-#define GF_MAIN_HOT(name, minb, hot)                                                           \
+#define GF_KERNELS(name, minb, hot, second)                                                    \
     __device__ int gf_main_##name(int argc, char **argv);                                     \
     static cudaError_t gf_launch_##name(void **args, unsigned grid, unsigned block, void *stream) \
     {                                                                                          \
-        return cudaLaunchCooperativeKernel((const void *)&gfd::program_kernel<gf_main_##name, minb, hot>, \
+        return cudaLaunchCooperativeKernel((const void *)&gfd::program_kernel<gf_main_##name, minb, hot, second>, \
                                            dim3(grid), dim3(block), args, 0, (cudaStream_t)stream); \
     }                                                                                          \
     static int gf_occ_##name(unsigned block)                                                   \
     {                                                                                          \
         int n = 0;                                                                             \
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                     \
-                &n, (const void *)&gfd::program_kernel<gf_main_##name, minb, hot>, (int)block, 0) != cudaSuccess) \
+                &n, (const void *)&gfd::program_kernel<gf_main_##name, minb, hot, second>, (int)block, 0) != cudaSuccess) \
             return -1;                                                                         \
         return n;                                                                              \
     }                                                                                          \
@@ -1098,10 +1133,21 @@ __global__ void __launch_bounds__(GF_BLOCK, MINB) region_kernel(gf_state *S)
         }                                                                                      \
         return cudaLaunchKernel((const void *)&gfd::region_kernel<gf_main_##name, minb>, dim3(grid), \
                                 dim3(block), args, 0, (cudaStream_t)stream);                   \
-    }                                                                                          \
+    }
+
+#define GF_MAIN_HOT(name, minb, hot)                                                           \
+    GF_KERNELS(name, minb, hot, false)                                                         \
     static const int gf_reg_##name =                                                           \
         gf_program_register(#name, gf_launch_##name, gf_occ_##name, gf_region_##name);        \
     __device__ int gf_main_##name
+
+/* GF_SECOND(name, second, minb, pick)(int argc, char **argv) { ... } defines the second kernel of program
+ * `name` (gf_program_second) */
+#define GF_SECOND(name, second, minb, pick)                                                    \
+    GF_KERNELS(second, minb, gfd::no_hot, true)                                                \
+    static const int gf_reg_##second =                                                         \
+        gf_program_second(#name, pick, gf_launch_##second, gf_occ_##second, gf_region_##second); \
+    __device__ int gf_main_##second
 
 #define GF_MAIN_BOUNDS(name, minb) GF_MAIN_HOT(name, minb, gfd::no_hot)
 

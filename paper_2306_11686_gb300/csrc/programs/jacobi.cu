@@ -4,82 +4,37 @@
  * grid written to a file.  Its serial twin in plain C with the real libc is
  * what a run must reproduce, bit for bit.
  */
-#include "../gf_device.cuh"
-#include "../gf_fastdiv.cuh"
-#include "../gf_intpipe.cuh"
+#include "jacobi.cuh"
 #include "../gf_fixsum.cuh"
 
 /*
- * One Jacobi sweep: the six-neighbour average of the interior into un, 0 on
- * the boundary, and the max residual |un - u| over the grid as a max
- * reduction.  The five neighbour adds keep the serial program's order; the
- * first INT_ADDS of them run on the integer pipe and the rest on the FP64
- * pipe (every one correctly rounded, so the split changes no bit of the
- * result, only which pipe does the work), as do the division by 6 and the
- * absolute value.  The flat index is split into (i, j, k) by multiplication
- * with an invariant-divisor magic number.
+ * The sweep for the grids that no fixed-point window suits, in the kernel that
+ * is compiled for the fixed-point sweep (2 blocks per SM): columns of
+ * JACOBI_SEG planes, every add on the FP64 pipe, and the loads of the next
+ * point on their way while one is computed, because 16 warps an SM do not hide
+ * them.  256^3 with values of both signs: 204 us (jacobi_sweep<0> 212 here;
+ * the FP64 pipe's six operations a point alone take 186); segments of 2, 4, 8
+ * and 16 planes 203.8, 204.2, 204.6 and 209.3; two points at a time 217; the
+ * first add on the integer pipe 205 to 233.
  */
-template <int INT_ADDS>
-__device__ int jacobi_sweep(const double *u, double *un, uint32_t nn, gf_udiv32 dn, uint64_t cells, double *res)
+#define JACOBI_SEG 4u
+static __device__ int jacobi_sweep_ahead(const double *u, double *un, uint32_t nn, gf_udiv32 dn, gf_udiv32 dsk,
+                                         double *res)
 {
     const uint32_t sk = nn * nn;
     return gf_reduce<double, GF_RED_MAX>(
-        0, (int64_t)cells, GF_SCHED_STATIC, 1,
-        [=](int64_t c64) -> double {
-            const uint32_t c = (uint32_t)c64;
-            /* i - 1, j - 1, k - 1 wrap to 2^32 - 1 at 0, so one unsigned
-             * compare of their maximum finds every boundary cell */
-            const uint32_t jk = dn.div(c), im1 = c - 1u - jk * nn;
-            const uint32_t k = dn.div(jk), jm1 = jk - 1u - k * nn;
-            if (max(im1, max(jm1, k - 1u)) >= nn - 2u) {
-                un[c] = 0.0;
-                return 0.0;
-            }
-            /* u is not written during the sweep: read-only loads, which may be
-             * issued ahead of the previous iteration's store to un */
-            const double nb[6] = {__ldg(u + c - 1),  __ldg(u + c + 1),  __ldg(u + c - nn),
-                                  __ldg(u + c + nn), __ldg(u + c - sk), __ldg(u + c + sk)};
-            double v = nb[0];
-#pragma unroll
-            for (int t = 1; t < 6; t++)
-                v = t <= INT_ADDS ? gf_dadd_int(v, nb[t]) : __dadd_rn(v, nb[t]);
-            v = gf_div6_int(v);               /* == v / 6.0, bit for bit */
-            un[c] = v;
-            return gf_fabs_int(__dadd_rn(v, -__ldg(u + c)));
-        },
-        res);
-}
-
-/*
- * The same sweep written with the k loop inside the parallel loop: work item
- * t is the column (i, j) over planes [k0, k0 + kseg), t = (k0 / kseg) * n^2 +
- * j * n + i, so consecutive items are consecutive i (coalesced).  Walking up
- * the column, the k - 1 and k neighbours of a point are the values loaded for
- * the previous point, so each point loads five values instead of seven, and
- * the index split and boundary test are paid once per column segment.  Every
- * point's arithmetic and its order are those of jacobi_sweep, so the grid
- * and the residual are the same bits.
- */
-template <int INT_ADDS>
-__device__ int jacobi_sweep_col(const double *u, double *un, uint32_t nn, gf_udiv32 dn, gf_udiv32 dsk, uint32_t kseg,
-                                double *res)
-{
-    const uint32_t sk = nn * nn;
-    const uint32_t nseg = (nn + kseg - 1) / kseg;
-    return gf_reduce<double, GF_RED_MAX>(
-        0, (int64_t)nseg * sk, GF_SCHED_STATIC, 1,
+        0, (int64_t)((nn + JACOBI_SEG - 1u) / JACOBI_SEG) * sk, GF_SCHED_STATIC, 1,
         [=](int64_t t64) -> double {
             const uint32_t t = (uint32_t)t64;
             const uint32_t seg = dsk.div(t), ij = t - seg * sk;
             const uint32_t j = dn.div(ij), im1 = ij - 1u - j * nn;
-            const uint32_t k0 = seg * kseg, k1 = min(k0 + kseg, nn);
+            const uint32_t k0 = seg * JACOBI_SEG, k1 = min(k0 + JACOBI_SEG, nn);
             double *o = un + ij;
             if (max(im1, j - 1u) >= nn - 2u) {            /* a boundary column */
                 for (uint32_t k = k0; k < k1; k++)
                     o[(size_t)k * sk] = 0.0;
                 return 0.0;
             }
-            const double *c = u + ij;
             uint32_t k = k0;
             if (k == 0) {                                  /* the bottom boundary plane */
                 o[0] = 0.0;
@@ -88,27 +43,33 @@ __device__ int jacobi_sweep_col(const double *u, double *un, uint32_t nn, gf_udi
             const uint32_t kend = min(k1, nn - 1u);
             long long best = 0;                            /* bits of the largest |un - u|, +0 to start */
             if (k < kend) {
-                double um = __ldg(c + (size_t)(k - 1) * sk), u0 = __ldg(c + (size_t)k * sk);
-                for (; k < kend; k++) {
-                    const double *p = c + (size_t)k * sk;
-                    const double up = __ldg(p + sk);
-                    const double nb[6] = {__ldg(p - 1), __ldg(p + 1), __ldg(p - nn), __ldg(p + nn), um, up};
-                    double v = nb[0];
-#pragma unroll
-                    for (int q = 1; q < 6; q++)
-                        v = q <= INT_ADDS ? gf_dadd_int(v, nb[q]) : __dadd_rn(v, nb[q]);
+                const double *p = u + ij + (size_t)k * sk;
+                o += (size_t)k * sk;
+                double um = __ldg(p - sk), u0 = __ldg(p);
+                double il = __ldg(p - 1), ir = __ldg(p + 1), jl = __ldg(p - nn), jr = __ldg(p + nn), up = __ldg(p + sk);
+                for (;;) {
+                    double il1, ir1, jl1, jr1, up1;
+                    const bool more = ++k < kend;
+                    if (more) {
+                        p += sk;
+                        il1 = __ldg(p - 1), ir1 = __ldg(p + 1), jl1 = __ldg(p - nn), jr1 = __ldg(p + nn);
+                        up1 = __ldg(p + sk);
+                    }
+                    double v = __dadd_rn(__dadd_rn(__dadd_rn(__dadd_rn(__dadd_rn(il, ir), jl), jr), um), up);
                     v = gf_div6_int(v);
-                    o[(size_t)k * sk] = v;
+                    *o = v;
                     /* |un - u| >= 0: its bits order as the values do; NaN is skipped, as the reduction does */
                     const long long b = __double_as_longlong(gf_fabs_int(__dadd_rn(v, -u0)));
                     if (b <= 0x7ff0000000000000ll && b > best)
                         best = b;
-                    um = u0;
-                    u0 = up;
+                    if (!more)
+                        break;
+                    o += sk;
+                    um = u0, u0 = up, up = up1, il = il1, ir = ir1, jl = jl1, jr = jr1;
                 }
             }
             if (k1 == nn && nn > 1)                        /* the top boundary plane */
-                o[(size_t)(nn - 1) * sk] = 0.0;
+                un[ij + (size_t)(nn - 1) * sk] = 0.0;
             return __longlong_as_double(best);
         },
         res);
@@ -423,11 +384,11 @@ struct jacobi_fix_body {
     }
 };
 
-/* grids from here on: a sweep of 96^3 takes 18.0 us on either path, of 112^3 16.9 against 24.7 us; smaller ones
- * would also pay for the sample's two regions (10 us) */
-#define JACOBI_FIX_CELLS (1u << 20)
 #define JACOBI_SAMPLE 32768
-/* a sample of the grid's values: their largest high word, and how many lie outside the window that starts at elow */
+#define JACOBI_TRIES 3       /* FP64 sweeps after which a grid that few values keep from a window goes over */
+/* a sample of the grid's values.  elow = 0: their largest high word, in red->out how many no window can hold
+ * (negative, infinite, NaN or above the highest) and, 2^16 each, how many are zero; else in red->out how many lie
+ * outside the window that starts at elow */
 static __device__ int jacobi_sample(const double *u, uint32_t cells, uint32_t elow, jacobi_red *red)
 {
     return gf_reduce<jacobi_red, GF_RED_MAX>(
@@ -439,6 +400,8 @@ static __device__ int jacobi_sample(const double *u, uint32_t cells, uint32_t el
             h ^= h >> 13;
             const uint64_t b = gf_ip_bits(__ldg(u + __umulhi(h, cells)));
             const uint32_t hi = (uint32_t)(b >> 32);
+            if (elow == 0u)
+                return jacobi_red{0ull, (int)hi, (hi >> 20 > GF_FIX_TOP ? 1u : 0u) + (b << 1 == 0ull ? 0x10000u : 0u)};
             return jacobi_red{0ull, (int)hi, b != 0ull && (hi >> 20) - elow > 8u ? 1u : 0u};
         },
         red);
@@ -446,18 +409,27 @@ static __device__ int jacobi_sample(const double *u, uint32_t cells, uint32_t el
 
 /* the lowest binade (biased exponent) of the fixed-point window that suits the grid u, 0 if none does: less
  * than one value in 4096 may lie outside it (each costs up to six points the FP64 path).  +0 lies in every
- * window; a sample of nothing else takes the one that ends at 2, and the first sweep sees what there is. */
-static __device__ uint32_t jacobi_window(const double *u, uint32_t cells, int *rc)
+ * window; a sample of nothing else takes the one that ends at 2, and the first sweep sees what there is.
+ * *fp64: the second kernel is the faster one for the grid: many values lie outside (of values uniform from 0 up to
+ * one in 256 does, and none after a sweep), or `tries` sweeps have found no window; a grid with many zeros gains
+ * nothing there. */
+static __device__ uint32_t jacobi_window(const double *u, uint32_t cells, int tries, bool *fp64, int *rc)
 {
     jacobi_red red{0ull, 0, 0u};
     *rc = jacobi_sample(u, cells, 0u, &red);
-    const uint32_t top = (uint32_t)red.hi >> 20;
-    if (!*rc && red.hi == 0 && red.out == 0u)
+    const uint32_t top = (uint32_t)red.hi >> 20, zeros = red.out >> 16;
+    uint32_t bad = red.out & 0xffffu;
+    *fp64 = false;
+    if (!*rc && zeros == JACOBI_SAMPLE && bad == 0u)
         return 1015u;
-    if (*rc || top < 13u || top > GF_FIX_TOP)
-        return 0u;
-    *rc = jacobi_sample(u, cells, top - 8u, &red);
-    return *rc || red.out > JACOBI_SAMPLE / 4096 ? 0u : top - 8u;
+    if (!*rc && bad <= JACOBI_SAMPLE / 4096 && top >= 13u && top <= GF_FIX_TOP) {
+        *rc = jacobi_sample(u, cells, top - 8u, &red);
+        bad = red.out;
+        if (!*rc && bad <= JACOBI_SAMPLE / 4096)
+            return top - 8u;
+    }
+    *fp64 = zeros <= JACOBI_SAMPLE / 8 && (bad > JACOBI_SAMPLE / 128 || tries >= JACOBI_TRIES);
+    return 0u;
 }
 
 /* segments of k for the fixed-point sweep: with r rounds of the warps' items there is room for r * warps / tiles
@@ -488,59 +460,58 @@ static __device__ jacobi_cut jacobi_make_cut(uint32_t nn, uint32_t warps)
  * a fresh grid from the device heap every sweep (old one freed after the
  * swap), the max residual over the interior fused into the sweep as a max
  * reduction, one printf per sweep, the final grid fwrite'd.  Without further
- * arguments a sweep runs on the FP32 pipe (jacobi_sweep_fix) while a window
+ * arguments a sweep runs on the FP32 pipe (jacobi_fix_body) while a window
  * of binades holds the grid's values, else on the FP64 pipe.  int_adds (0..5)
  * asks for jacobi_sweep with that many of the five neighbour adds on the
  * integer pipe; kseg > 0 runs it as columns of kseg planes
  * (jacobi_sweep_col) instead of one parallel iteration per point.
+ *
+ * Two kernels: jacobi_fix_body wants 104 registers, 2 resident blocks per SM,
+ * and the FP64-pipe sweeps want 4 (256^3, uniform data: 173 us with one
+ * integer add at 4 blocks per SM, 217 at 2).  The first kernel has the
+ * fixed-point sweep, and FP64 sweeps for small grids, for the time between two
+ * samples and for grids with many zeros.  The second one has the sweeps that
+ * the options ask for, and takes over the grids that no window suits.
  */
-/* 2 resident blocks per SM: jacobi_fix_body wants 104 registers.  The FP64-pipe sweeps lose by it (256^3: 209 us
- * with no integer add against 173 with one at 4 blocks per SM), so they keep only the grids that no window suits
- * and the small ones.  The fixed sweep is part of the worker loop: behind the trampoline pointer it took 111 us. */
+/* The fixed sweep is part of the worker loop: behind the trampoline pointer it took 111 us. */
 using jacobi_hot = gfd::hot_reduce<jacobi_red, GF_RED_MAX, jacobi_fix_body>;
 GF_MAIN_HOT(jacobi, 2, jacobi_hot)(int argc, char **argv)
 {
-    if (argc < 4)
+    jacobi_job job;
+    if (!jacobi_parse(argc, argv, &job))
         return 2;
-    const long long n = gf_atoll(argv[1]);
-    const int sweeps = (int)gf_atoll(argv[2]);
-    const int int_adds = argc > 4 ? (int)gf_atoll(argv[4]) : 1;
-    const long long kseg = argc > 5 ? gf_atoll(argv[5]) : 0;
-    const double *u0 = (const double *)gf_buffer(0);
-    const uint64_t cells = (uint64_t)n * n * n;
-    if (n < 1 || n > 1290 || !u0 || gf_buffer_bytes(0) < cells * 8 || int_adds < 0 || int_adds > 5 || kseg < 0 ||
-        kseg > n)
-        return 2;
-    const uint32_t nn = (uint32_t)n;
-    const double *u = u0;
     double *owned = nullptr;
+    const uint32_t nn = job.nn, cells = (uint32_t)job.cells;
     /* the index split's magic numbers: loop invariants, made once */
     const gf_udiv32 dn = gf_udiv32::make(nn), dsk = gf_udiv32::make(nn * nn);
     const jacobi_cut cut = jacobi_make_cut(nn, (uint32_t)(gfd::s_st->nworkers >> 5));
     const gf_udiv32 dt = gf_udiv32::make(cut.tiles);
     uint32_t elow = 0u;                            /* window of the fixed-point sweeps, 0: not known */
     int ask = 0, pause = 0;                        /* sweeps until the grid is sampled for a window (again) */
-    for (int s = 1; s <= sweeps; s++) {
-        double *un = (double *)gf_malloc(cells * sizeof(double));
-        if (!un) {
-            gf_printf("jacobi: out of device heap at sweep %d\n", s);
-            return 4;
-        }
+    int tries = 0;                                 /* sweeps without a window */
+    for (int s = 1; s <= job.sweeps; s++) {
+        const double *u = owned ? owned : job.u0;
         double res = 0.0;
         int rc = 0;
-        if (argc <= 4 && cells >= JACOBI_FIX_CELLS && !elow && ask-- == 0) {
-            elow = jacobi_window(u, (uint32_t)cells, &rc);
+        if (cells >= JACOBI_FIX_CELLS && !elow && ask-- == 0) {
+            bool fp64;
+            elow = jacobi_window(u, cells, tries, &fp64, &rc);
             ask = pause;
             pause = min(2 * pause + 1, 15);
+            if (rc)
+                return 10;
+            if (fp64 && gf_second_kernel((uint64_t)s, (uint64_t)owned))
+                return 0;
         }
-        if (rc) {
-            ;
-        } else if (elow) {
+        double *un = jacobi_grid(job, s);
+        if (!un)
+            return 4;
+        if (elow) {
             jacobi_red red, rest{0ull, 0, 0u};
             rc = gf_reduce<jacobi_red, GF_RED_MAX>(0, (int64_t)cut.warps * 32, GF_SCHED_STATIC, 1,
                                                    jacobi_fix_body{u, un, nn, elow, dn, dt, cut}, &red);
             if (!rc && red.out)
-                rc = jacobi_rest(u, un, nn, (uint32_t)cells, &rest);
+                rc = jacobi_rest(u, un, nn, cells, &rest);
             res = __longlong_as_double((long long)max(red.res, rest.res));
             const uint32_t hi = (uint32_t)max(red.hi, rest.hi), top = hi >> 20;
             if (red.out > cells / 64) {            /* the window does not suit: the FP64 pipe for a while */
@@ -551,47 +522,14 @@ GF_MAIN_HOT(jacobi, 2, jacobi_hot)(int argc, char **argv)
                     elow = top < 13u || top > GF_FIX_TOP ? 0u : top - 8u;
                 ask = pause = 0;
             }
-        } else if (argc <= 4) {
-            rc = jacobi_sweep<0>(u, un, nn, dn, cells, &res);
-        } else if (kseg > 0) {
-            const uint32_t ks = (uint32_t)kseg;
-            switch (int_adds) {
-            case 0: rc = jacobi_sweep_col<0>(u, un, nn, dn, dsk, ks, &res); break;
-            case 1: rc = jacobi_sweep_col<1>(u, un, nn, dn, dsk, ks, &res); break;
-            case 2: rc = jacobi_sweep_col<2>(u, un, nn, dn, dsk, ks, &res); break;
-            case 3: rc = jacobi_sweep_col<3>(u, un, nn, dn, dsk, ks, &res); break;
-            case 4: rc = jacobi_sweep_col<4>(u, un, nn, dn, dsk, ks, &res); break;
-            default: rc = jacobi_sweep_col<5>(u, un, nn, dn, dsk, ks, &res); break;
-            }
         } else {
-            switch (int_adds) {
-            case 0: rc = jacobi_sweep<0>(u, un, nn, dn, cells, &res); break;
-            case 1: rc = jacobi_sweep<1>(u, un, nn, dn, cells, &res); break;
-            case 2: rc = jacobi_sweep<2>(u, un, nn, dn, cells, &res); break;
-            case 3: rc = jacobi_sweep<3>(u, un, nn, dn, cells, &res); break;
-            case 4: rc = jacobi_sweep<4>(u, un, nn, dn, cells, &res); break;
-            default: rc = jacobi_sweep<5>(u, un, nn, dn, cells, &res); break;
-            }
+            rc = cells >= JACOBI_FIX_CELLS ? jacobi_sweep_ahead(u, un, nn, dn, dsk, &res)
+                                           : jacobi_sweep<0>(u, un, nn, dn, cells, &res);
+            tries++;
         }
         if (rc)
             return 10;
-        gf_printf("%d %.17g\n", s, res);
-        if (owned)
-            gf_free(owned);
-        owned = un;
-        u = un;
+        jacobi_swap(s, res, un, &owned);
     }
-    if (argv[3][0] == '-' && argv[3][1] == 0) {      /* "-": keep the grid, write nothing (profiling) */
-        if (owned)
-            gf_free(owned);
-        return 0;
-    }
-    GF_FILE f = gf_fopen(argv[3], "wb");
-    if (!f)
-        return 3;
-    const size_t w = gf_fwrite(u, sizeof(double), (size_t)cells, f);
-    gf_fclose(f);
-    if (owned)
-        gf_free(owned);
-    return w == cells ? 0 : 3;
+    return jacobi_write(job, owned);
 }

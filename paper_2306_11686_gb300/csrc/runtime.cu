@@ -56,6 +56,13 @@ struct ProgEntry {
     gf_occ_fn occ;
     gf_launch_fn region;    /* the program's region kernel (kernel split) */
 };
+struct SecondEntry {
+    std::string name;       /* the program's */
+    gf_pick_fn pick;
+    gf_launch_fn launch;
+    gf_occ_fn occ;
+    gf_launch_fn region;
+};
 static std::mutex &reg_mu()
 {
     static std::mutex m;
@@ -67,12 +74,27 @@ static std::vector<ProgEntry> &registry()
     return r;
 }
 
+static std::vector<SecondEntry> &seconds()
+{
+    static std::vector<SecondEntry> r;
+    return r;
+}
+
 extern "C" __attribute__((visibility("default"))) int gf_program_register(const char *name, gf_launch_fn launch,
                                                                            gf_occ_fn occ, gf_launch_fn region)
 {
     std::lock_guard<std::mutex> g(reg_mu());
     registry().push_back({name, launch, occ, region});
     return (int)registry().size() - 1;
+}
+
+extern "C" __attribute__((visibility("default"))) int gf_program_second(const char *name, gf_pick_fn pick,
+                                                                         gf_launch_fn launch, gf_occ_fn occ,
+                                                                         gf_launch_fn region)
+{
+    std::lock_guard<std::mutex> g(reg_mu());
+    seconds().push_back({name, pick, launch, occ, region});
+    return GF_OK;
 }
 
 /* ------------------------------------------------------------------ context */
@@ -586,6 +608,15 @@ extern "C" GF_API int gf_rpc_register(gf_ctx *c, uint32_t opcode, gf_host_fn fn,
     return c->server.register_user(opcode, fn, user);
 }
 
+static int resident(gf_occ_fn occ, uint32_t *per_sm)
+{
+    const int n = occ(GF_BLOCK_THREADS);
+    if (n < 1)
+        return GF_ECUDA;
+    *per_sm = (uint32_t)std::min(n, GF_MAX_BLOCKS_PER_SM);
+    return GF_OK;
+}
+
 static int occupancy(gf_ctx *c, gf_program prog, uint32_t *per_sm)
 {
     ProgEntry pe;
@@ -595,11 +626,7 @@ static int occupancy(gf_ctx *c, gf_program prog, uint32_t *per_sm)
             return GF_ENOENT;
         pe = registry()[prog];
     }
-    int occ = pe.occ(GF_BLOCK_THREADS);
-    if (occ < 1)
-        return GF_ECUDA;
-    *per_sm = (uint32_t)std::min(occ, GF_MAX_BLOCKS_PER_SM);
-    return GF_OK;
+    return resident(pe.occ, per_sm);
 }
 
 extern "C" GF_API int gf_grid_info(gf_ctx *c, gf_program prog, uint32_t *sms, uint32_t *per_sm)
@@ -714,21 +741,42 @@ extern "C" GF_API int gf_launch_q(gf_ctx *c, gf_program prog, int argc, const ch
         return GF_EINVAL;
     *out = nullptr;
     ProgEntry pe;
+    SecondEntry pe2 = {};
     {
         std::lock_guard<std::mutex> g(reg_mu());
         if (prog < 0 || (size_t)prog >= registry().size())
             return GF_ENOENT;
         pe = registry()[prog];
+        for (const SecondEntry &e : seconds())
+            if (e.name == pe.name)
+                pe2 = e;
     }
-    uint32_t per_sm = 0;
-    int rc = occupancy(c, prog, &per_sm);
+    uint32_t per_sm = 0, per_sm2 = 0;
+    int rc = resident(pe.occ, &per_sm);
+    if (rc == GF_OK && pe2.pick)
+        rc = resident(pe2.occ, &per_sm2);
     if (rc)
         return rc;
-    const uint32_t full = per_sm * (uint32_t)c->nsm;
+    const uint32_t sms = (uint32_t)c->nsm;
     if (!grid)
-        grid = c->cfg.grid ? c->cfg.grid : std::max<uint32_t>(1, full / c->cfg.max_programs);
-    if (grid > full || grid > (uint32_t)c->nsm * GF_MAX_BLOCKS_PER_SM)
+        grid = c->cfg.grid;
+    /* a grid larger than the first kernel's residency takes the second kernel, if that one has room for it */
+    int kernels = pe2.pick ? pe2.pick(argc, argv) : GF_FIRST_ONLY;
+    if (pe2.pick && grid > per_sm * sms)
+        kernels = GF_SECOND_ONLY;
+    if (kernels == GF_SECOND_ONLY) {
+        pe.launch = pe2.launch;
+        pe.region = pe2.region;
+        per_sm = per_sm2;
+    }
+    if (c->cfg.split_regions && kernels == GF_BOTH)
+        kernels = GF_FIRST_ONLY;         /* region kernels belong to one program kernel */
+    const uint32_t full = per_sm * sms;
+    if (!grid)
+        grid = std::max<uint32_t>(1, full / c->cfg.max_programs);
+    if (grid > full || grid > sms * GF_MAX_BLOCKS_PER_SM)
         return GF_EINVAL;
+    const uint32_t grid2 = (uint32_t)((uint64_t)grid * per_sm2 / per_sm);      /* the same share of the GPU */
     /* kernel split: the program kernel is one block (the initial thread's);
      * regions get the grid, less the block the program kernel holds */
     uint32_t region_grid = 0;
@@ -798,6 +846,8 @@ extern "C" GF_API int gf_launch_q(gf_ctx *c, gf_program prog, int argc, const ch
         s.buf_bytes[k] = bufs[k].bytes;
     }
     s.nbufs = (uint32_t)nbufs;
+    s.second = kernels == GF_SECOND_ONLY ? 1u : 0u;
+    s.second_follows = kernels == GF_BOTH ? 1u : 0u;
     if ((rc = inst_start(c, in, h->stream, grid, (uint32_t)need)) != GF_OK)
         return bail(rc);
     int a_argc = argc;
@@ -805,6 +855,8 @@ extern "C" GF_API int gf_launch_q(gf_ctx *c, gf_program prog, int argc, const ch
     gf_state *a_state = in->d_state;
     void *args[3] = {&a_state, &a_argc, &a_argv};
     cudaError_t le = pe.launch(args, grid, GF_BLOCK_THREADS, h->stream);
+    if (le == cudaSuccess && kernels == GF_BOTH)
+        le = pe2.launch(args, grid2, GF_BLOCK_THREADS, h->stream);
     if (le != cudaSuccess || cudaEventRecord(in->ev_done, h->stream) != cudaSuccess) {
         fprintf(stderr, "gf: launch of %s failed: %s\n", pe.name.c_str(), cudaGetErrorString(le));
         return bail(GF_ECUDA);

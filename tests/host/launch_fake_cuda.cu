@@ -13,6 +13,7 @@
  *            gives the instance back only when that kernel has run
  *   split    the state of a program whose regions are kernels of their own
  *            counts the threads of the region kernel as workers
+ *   second   which kernels a launch of a program with two takes, on what grids
  */
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -255,11 +256,71 @@ static bool split()
     return true;
 }
 
+static std::string launched;
+static cudaError_t first_launch(void **, unsigned grid, unsigned, void *)
+{
+    launched += "first " + std::to_string(grid) + " ";
+    return cudaSuccess;
+}
+static cudaError_t second_launch(void **, unsigned grid, unsigned, void *)
+{
+    launched += "second " + std::to_string(grid) + " ";
+    return cudaSuccess;
+}
+static int second_occ(unsigned) { return 4; }
+static int by_argc(int argc, const char *const *)
+{
+    return argc == 0 ? GF_BOTH : argc == 1 ? GF_SECOND_ONLY : GF_FIRST_ONLY;
+}
+
+static bool second()
+{
+    gf_program_second("two", by_argc, second_launch, second_occ, prog_launch);
+    const int p = gf_program_register("two", first_launch, prog_occ, prog_launch);
+    const struct {
+        int argc;
+        uint32_t programs, grid, split;
+        const char *want;              /* launches, then the state's second and second_follows */
+    } cases[] = {
+        {0, 1, 0, 0, "first 304 second 608 0 1"}, {1, 1, 0, 0, "second 608 1 0"},   {2, 1, 0, 0, "first 304 0 0"},
+        {0, 4, 0, 0, "first 76 second 152 0 1"},  {1, 4, 0, 0, "second 152 1 0"},   {0, 1, 100, 0, "first 100 second 200 0 1"},
+        {1, 1, 100, 0, "second 100 1 0"},         {0, 1, 400, 0, "second 400 1 0"}, {2, 1, 608, 0, "second 608 1 0"},
+        {0, 1, 609, 0, "refused"},                {1, 1, 609, 0, "refused"},        {0, 1, 0, 1, "first 1 0 0"},
+        {1, 1, 0, 1, "second 1 1 0"},
+    };
+    const char *argv[2] = {"two", "x"};
+    for (const auto &t : cases) {
+        gf_config cf = config();
+        cf.max_programs = t.programs;
+        cf.split_regions = t.split;
+        cf.server_threads = 1;
+        gf_ctx *c = nullptr;
+        gf_handle *h = nullptr;
+        int ec = 0;
+        if (gf_init(&cf, &c))
+            return false;
+        launched.clear();
+        const int rc = gf_launch(c, p, t.argc, argv, nullptr, 0, nullptr, t.grid, &h);
+        std::string got = rc == GF_EINVAL ? "refused" : launched;
+        if (rc == GF_OK) {
+            got += std::to_string(h->inst->h_init()->second) + " " + std::to_string(h->inst->h_init()->second_follows);
+            gf_wait(h, &ec, 0);
+        }
+        if (got != t.want) {
+            printf("argc %d programs %u grid %u split %u: %s, not %s\n", t.argc, t.programs, t.grid, t.split, got.c_str(),
+                   t.want);
+            return false;
+        }
+        gf_finalize(c);
+    }
+    return true;
+}
+
 int main(int argc, char **argv)
 {
     fake::arg_bytes = sizeof(ResetArgs);
     const std::string s = argc > 1 ? argv[1] : "";
-    const bool ok = s == "reset" ? reset() : s == "failed" ? failed() : s == "split" && split();
+    const bool ok = s == "reset" ? reset() : s == "failed" ? failed() : s == "split" ? split() : s == "second" && second();
     printf("%s%s\n", fake::trouble.c_str(), ok && fake::trouble.empty() ? "OK" : "FAILED");
     return ok && fake::trouble.empty() ? 0 : 1;
 }

@@ -1,7 +1,8 @@
 """A launch's host side with a fake CUDA runtime (no GPU): what the reset
 kernel writes lies inside the instance's allocations, and an instance goes to
 the next program only when that kernel has run, also where a launch fails, and
-a program's state counts the workers that its regions have."""
+a program's state counts the workers that its regions have, and a program with
+two kernels gets the ones that it asks for."""
 import os
 import subprocess
 
@@ -20,7 +21,7 @@ def launch_bin(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["reset", "failed", "split"])
+@pytest.mark.parametrize("scenario", ["reset", "failed", "split", "second"])
 def test_launch_scenario(launch_bin, scenario):
     p = subprocess.run([launch_bin, scenario], capture_output=True, text=True, timeout=120)
     assert p.returncode == 0, p.stdout + p.stderr
