@@ -260,7 +260,6 @@ struct jacobi_fix_body {
                 continue;
             const double *p = u + (size_t)k * sk;
             double *o = un + (size_t)k * sk;
-            const uint32_t kfirst = k;
             uint32_t left0 = 0u, left1 = 0u, left = 0u;     /* first and last plane with points left out, this lane's count */
             gf_fix3 m[R], c[R], s[R];                  /* planes k - 1 and k in chunks; the sums */
             /* a ring slot holds the centre rows of a plane and the halo rows of the plane below it */
@@ -277,14 +276,12 @@ struct jacobi_fix_body {
             fetch(ring + JACOBI_SLOT, p + sk, true);
             copy_commit();
             const double *ahead = p + 2 * (size_t)sk;  /* the next plane to fetch, up to kend */
-            uint32_t ka = k + 2u;
 #pragma unroll
             for (int d = 2; d <= JACOBI_AHEAD; d++) {
-                if (ka <= kend)
+                if (k + d <= kend)
                     fetch(ring + d * JACOBI_SLOT, ahead, true);
                 copy_commit();
                 ahead += sk;
-                ka++;
             }
 #pragma unroll
             for (int q = 0; q < R; q++)
@@ -357,11 +354,10 @@ struct jacobi_fix_body {
                         left1 = k;
                     }
                 }
-                if (ka <= kend)                        /* into the slot of plane k, which is done */
+                if (k + (JACOBI_AHEAD + 1) <= kend)    /* into the slot of plane k, which is done */
                     fetch(here, ahead, true);
                 copy_commit();
                 ahead += sk;
-                ka++;
                 o += sk;
                 here = next;
                 next += JACOBI_SLOT;
