@@ -274,7 +274,8 @@ template <> struct acc<double, GF_RED_SUM> {
     __device__ void add(double x)
     {
         double t = __dadd_rn(s, x);
-        if (fabs(s) >= fabs(x))
+        /* |s| >= |x|, on the integer pipe */
+        if (gf_ip_bits(s) << 1 >= gf_ip_bits(x) << 1)
             c = __dadd_rn(c, __dadd_rn(__dadd_rn(s, -t), x));
         else
             c = __dadd_rn(c, __dadd_rn(__dadd_rn(x, -t), s));
@@ -389,10 +390,10 @@ template <> struct part<double, GF_RED_SUM> {
             if (--room == 0u)
                 fold();
         } else {
-            w.add_out(x, [&](double y) { a.add(y); });
+            w.add_out(x, [&](double y) { a.add(y); }, room);
         }
     }
-    /* four values with one test where all lie in the window */
+    /* four values with one test where all lie in the window; the first four open it for their largest */
     __device__ __forceinline__ void add4(double2 p, double2 q)
     {
         const uint32_t p0 = w.place(p.x), p1 = w.place(p.y), p2 = w.place(q.x), p3 = w.place(q.y);
@@ -405,10 +406,11 @@ template <> struct part<double, GF_RED_SUM> {
             if (room == 0u)
                 fold();
         } else {
-            add(p.x);
-            add(p.y);
-            add(q.x);
-            add(q.y);
+            if (!w.base)                       /* place() is the exponent */
+                w.open(max(max(p0, p1), max(p2, p3)));
+#pragma unroll 1
+            for (int k = 0; k < 4; k++)
+                add(k == 0 ? p.x : k == 1 ? p.y : k == 2 ? q.x : q.y);
         }
     }
     __device__ void tree(int width);
