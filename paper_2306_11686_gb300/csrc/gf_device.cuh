@@ -68,7 +68,7 @@ __shared__ uint32_t s_kr;                  /* 1 outside a program's persistent k
 __shared__ uint64_t s_red[GF_MAX_WARPS][2];/* per-warp reduction partials               */
 __shared__ uint32_t s_sum[GF_MAX_WARPS][5];/* ... of a double sum: the integer, its window */
 __shared__ uint64_t s_xfer[GF_MAX_WARPS][32]; /* per-warp lane hand-off (heap, rpc)    */
-__shared__ unsigned long long s_heap_high; /* the most live heap bytes this block has seen  */
+__shared__ long long s_heap_high;          /* the most live heap bytes this block has seen  */
 /* the initial thread's own bookkeeping, kept in its block's shared memory so
  * that its serial part pays no global-memory round trip for it: */
 __shared__ uint32_t s_done_target;         /* blocks done when the current region ends   */

@@ -148,28 +148,37 @@ static __device__ __forceinline__ bool heap_push1(gf_heap *H, uint32_t sm, uint3
  * pairs of 16 B to 64 KiB, 2.4 ms counted like this (2.1 with every step of
  * this file; what is left are the stacks' round trips, about 20 us a warp's
  * pair, and the compare-and-swaps that 16 warps an SM lose to each other).
- * Allocations are counted before they are made, so their atomics
- * overlap the search (an allocation that fails is taken back, and can show in
- * a high-water reading meanwhile).
+ * Blocks are counted once they are granted, and no longer from when their
+ * free begins, so the count never exceeds what is live.  What was live at most
+ * was live before some free or at the program's end: frees take the readings,
+ * whose round trip overlaps the push, and the host looks at the last one.
+ * (With a reading at every malloc, whose caller waits for it, the pairs above
+ * took 5% longer; counting before the search hid that and showed requests
+ * that then failed.)
  */
 static __device__ __forceinline__ void count_alloc(gf_heap *H, uint32_t active, uint32_t bytes)
 {
     const uint32_t sum = __reduce_add_sync(active, bytes);
     if (lane_id() == __ffs(active) - 1) {
-        const unsigned long long live = atomicAdd((unsigned long long *)&H->live_bytes, (unsigned long long)sum) + sum;
+        atomicAdd((unsigned long long *)&H->live_bytes, (unsigned long long)sum);
         atomicAdd((unsigned long long *)&H->n_alloc, (unsigned long long)__popc(active));
-        if (live > s_heap_high) {      /* this block has not seen as much: most readings stop here */
-            s_heap_high = live;
-            atomicMax((unsigned long long *)&H->high_water, live);
-        }
     }
 }
-static __device__ __forceinline__ void count_free(gf_heap *H, uint32_t active, uint32_t bytes)
+/* in one lane: the live bytes before these frees (signed: a lane that runs ahead can be counted before the one
+ * that counts its malloc), else 0 */
+static __device__ __forceinline__ long long count_free(gf_heap *H, uint32_t active, uint32_t bytes)
 {
     const uint32_t sum = __reduce_add_sync(active, bytes), n = __popc(__ballot_sync(active, bytes != 0u));
-    if (n && lane_id() == __ffs(active) - 1) {
-        atomicAdd((unsigned long long *)&H->n_free, (unsigned long long)n);
-        atomicAdd((unsigned long long *)&H->live_bytes, 0ull - sum);
+    if (!n || lane_id() != __ffs(active) - 1)
+        return 0;
+    atomicAdd((unsigned long long *)&H->n_free, (unsigned long long)n);
+    return (long long)atomicAdd((unsigned long long *)&H->live_bytes, 0ull - sum);
+}
+static __device__ __forceinline__ void note_live(gf_heap *H, long long live)
+{
+    if (live > s_heap_high) {          /* this block has not seen as much: most readings stop here */
+        s_heap_high = live;
+        atomicMax((long long *)&H->high_water, live);
     }
 }
 
@@ -541,7 +550,6 @@ static __device__ __forceinline__ void *gf_malloc_body(size_t n)
     }
     const uint32_t cls = gfd::size_class(n ? n : 1);
     const uint32_t lane = gfd::lane_id(), warp = threadIdx.x >> 5;
-    gfd::count_alloc(H, __activemask(), 16u << cls);
     const uint32_t sm = gfd::smid() % GF_MAX_SM;
     uint64_t *out = gfd::s_xfer[warp];
     /* every lane: its own stack */
@@ -566,11 +574,10 @@ static __device__ __forceinline__ void *gf_malloc_body(size_t n)
         if (!p)                        /* no fresh slab: other stacks before failing */
             p = gfd::heap_steal1(H, sm, cls, lane);
     }
-    if (!p) {                          /* counted above, not granted */
-        atomicAdd((unsigned long long *)&H->n_alloc, ~0ull);
+    if (p)
+        gfd::count_alloc(H, __activemask(), 16u << cls);
+    else
         atomicAdd((unsigned long long *)&H->n_fail, 1ull);
-        atomicAdd((unsigned long long *)&H->live_bytes, 0ull - (16ull << cls));
-    }
     return (void *)p;
 }
 
@@ -593,8 +600,9 @@ static __device__ __forceinline__ void gf_free_body(void *p)
             small = true;
         }
     }
-    gfd::count_free(H, __activemask(), small ? 16u << cls : 0u);
+    const long long live = gfd::count_free(H, __activemask(), small ? 16u << cls : 0u);
     if (!small) {
+        gfd::note_live(H, live);
         if (a >= H->large_base && a < H->large_base + H->large_bytes) {
             const uint32_t np = gfd::large_release(H, a, S->timeout_ns);
             if (np) {
@@ -614,6 +622,7 @@ static __device__ __forceinline__ void gf_free_body(void *p)
         atomicAdd((unsigned long long *)&H->n_free, ~0ull);
         atomicAdd((unsigned long long *)&H->live_bytes, 16ull << cls);
     }
+    gfd::note_live(H, live);
 }
 
 /* malloc / free; the initial thread's time in them is counted (st_heap_ns),

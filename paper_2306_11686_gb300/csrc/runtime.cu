@@ -1116,7 +1116,7 @@ extern "C" GF_API int gf_wait(gf_handle *h, int *exit_code, int64_t timeout_ns)
         st.heap_fail = f.heap.n_fail;
         st.heap_bad_free = f.heap.n_bad_free;
         st.heap_live_bytes = f.heap.live_bytes;
-        st.heap_high_water = f.heap.high_water;
+        st.heap_high_water = std::max(f.heap.high_water, f.heap.live_bytes);
         st.main_ns = f.t_main_end > f.t_main_start ? f.t_main_end - f.t_main_start : 0;
         st.host_slots = c->server.stats.slots;
         st.host_records = c->server.stats.records;
