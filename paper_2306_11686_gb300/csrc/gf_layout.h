@@ -197,10 +197,6 @@ typedef struct gf_state {
     uint64_t buf_bytes[GF_MAX_BUFS];
     uint32_t nbufs;
     uint32_t split;            /* 1: regions run as host-launched kernels (the paper's split) */
-    uint32_t second_follows;   /* the program's second kernel is queued behind the first       */
-    uint32_t second;           /* 1: the second kernel runs main, 2: it continues (second_arg) */
-    uint32_t epoch0, done0;    /* where a continuing kernel's epoch and done_blocks start      */
-    uint64_t second_arg[2];
     /* results written by the device */
     int32_t exit_code, error, main_done;
     uint64_t st_calls[GF_NSTAT];  /* RPC calls per opcode (lane records)              */
@@ -217,6 +213,10 @@ typedef struct gf_state {
     uint64_t lat_hist[GF_LAT_BUCKETS];  /* RPC round trips (claim -> host done), lane records */
     uint32_t rand_words[40];      /* rand() state of the program (device libc)        */
     gf_heap heap;
+    uint32_t second_follows;   /* the program's second kernel is queued behind the first       */
+    uint32_t second;           /* 1: the second kernel runs main, 2: it continues (second_arg) */
+    uint32_t epoch0, done0;    /* where a continuing kernel's epoch and done_blocks start      */
+    uint64_t second_arg[2];
 } gf_state;
 
 #endif
