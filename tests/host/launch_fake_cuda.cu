@@ -13,6 +13,8 @@
  *            gives the instance back only when that kernel has run
  *   split    the state of a program whose regions are kernels of their own
  *            counts the threads of the region kernel as workers
+ *   clear    the heap's metadata and the format cache are zero when the program
+ *            starts, in contexts for one program and for several
  *   second   which kernels a launch of a program with two takes, on what grids
  */
 #include <cuda_runtime.h>
@@ -95,6 +97,14 @@ template <class T> cudaError_t is(T *p, T v)
     *p = v;
     return cudaSuccess;
 }
+cudaError_t clear(void *d, size_t n)
+{
+    if (!inside((uint64_t)d, n))
+        trouble += "a memset reaches past its allocation\n";
+    else
+        memset(d, 0, n);
+    return cudaSuccess;
+}
 cudaError_t dev_pointer(cudaPointerAttributes *a)
 {
     memset(a, 0, sizeof *a);
@@ -121,6 +131,7 @@ cudaError_t dev_pointer(cudaPointerAttributes *a)
 #define cudaStreamSynchronize(s) fake::drain(s)
 #define cudaMemcpyAsync(d, s, n, k, st) fake::copy((void *)(d), (const void *)(s), n, st)
 #define cudaLaunchKernel(f, g, b, args, shm, s) fake::launch(args, s)
+#define cudaMemsetAsync(d, v, n, s) fake::clear(d, n)
 #define cudaSetDevice(d) cudaSuccess
 #define cudaGetDevice(d) fake::is(d, 0)
 #define cudaDeviceGetAttribute(v, a, d) fake::is(v, 152)
@@ -256,6 +267,48 @@ static bool split()
     return true;
 }
 
+static bool clear()
+{
+    const int p = prog();
+    for (uint32_t programs : {1u, 3u}) {
+        gf_config cf = config();
+        cf.max_programs = programs;
+        cf.heap_bytes = 3 << 20;
+        gf_ctx *c = nullptr;
+        if (gf_init(&cf, &c))
+            return false;
+        for (int turn = 0; turn < 2; turn++) {
+            gf_handle *h = nullptr;
+            int ec = 0;
+            for (Instance *in : c->inst)
+                for (void *a : {in->d_meta, in->d_heads, in->d_cur, in->d_lsize, in->d_fmt})
+                    memset(a, 0x5a, fake::mem[(uint64_t)a]);
+            if (gf_launch(c, p, 0, nullptr, nullptr, 0, nullptr, 0, &h))
+                return false;
+            fake::drain(h->stream);
+            const Instance *in = h->inst;
+            const struct {
+                const void *at;
+                size_t n;
+            } want[] = {{in->d_meta, in->nslabs * 16ull},
+                        {in->d_heads, (size_t)GF_MAX_SM * GF_HEAP_NCLASS * GF_HEAP_LANES * 8},
+                        {in->d_cur, (size_t)GF_MAX_SM * GF_HEAP_NCLASS * 4},
+                        {in->d_lsize, in->npages * 4ull},
+                        {in->d_fmt, cf.fmt_cache * 8ull}};
+            for (const auto &w : want)
+                for (size_t k = 0; k < w.n; k++)
+                    if (((const char *)w.at)[k]) {
+                        printf("programs %u: a byte is left\n", programs);
+                        return false;
+                    }
+            if (gf_wait(h, &ec, 0))
+                return false;
+        }
+        gf_finalize(c);
+    }
+    return true;
+}
+
 static std::string launched;
 static cudaError_t first_launch(void **, unsigned grid, unsigned, void *)
 {
@@ -320,7 +373,7 @@ int main(int argc, char **argv)
 {
     fake::arg_bytes = sizeof(ResetArgs);
     const std::string s = argc > 1 ? argv[1] : "";
-    const bool ok = s == "reset" ? reset() : s == "failed" ? failed() : s == "split" ? split() : s == "second" && second();
+    const bool ok = s == "reset" ? reset() : s == "failed" ? failed() : s == "split" ? split() : s == "clear" ? clear() : s == "second" && second();
     printf("%s%s\n", fake::trouble.c_str(), ok && fake::trouble.empty() ? "OK" : "FAILED");
     return ok && fake::trouble.empty() ? 0 : 1;
 }

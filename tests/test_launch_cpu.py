@@ -21,7 +21,7 @@ def launch_bin(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["reset", "failed", "split", "second"])
+@pytest.mark.parametrize("scenario", ["reset", "failed", "split", "clear", "second"])
 def test_launch_scenario(launch_bin, scenario):
     p = subprocess.run([launch_bin, scenario], capture_output=True, text=True, timeout=120)
     assert p.returncode == 0, p.stdout + p.stderr
