@@ -76,8 +76,9 @@ static __device__ int jacobi_sweep_ahead(const double *u, double *un, uint32_t n
 }
 
 /* What a fixed-point sweep reduces: the largest |un - u| (its bits, NaN left
- * out), the largest high word of a new value (the next sweep's window) and
- * the number of points left out. */
+ * out), the largest high word among the old values of the planes that could
+ * raise it (a sample, from which the next sweep's window is taken) and the
+ * number of points left out. */
 struct jacobi_red {
     unsigned long long res;
     int hi;
@@ -203,8 +204,8 @@ struct jacobi_cut {
  *
  * What bounds it: issue slots and the integer pipe (142 warp instructions per
  * 30 points, 58 of them integer; 69% of the issue slots and 56% of the integer
- * pipe busy, 0.24 GB of DRAM traffic a sweep).  A sweep of 256^3 takes 101 us
- * against 173 us for jacobi_sweep<1> at 4 blocks per SM (the FP64 pipe's 5
+ * pipe busy, 0.24 GB of DRAM traffic a sweep).  A sweep of 256^3 takes 104 us
+ * (102.5 if sums of zeros were left out) against 173 us for jacobi_sweep<1> at 4 blocks per SM (the FP64 pipe's 5
  * operations a point alone take 155 us).  Measured for this layout in a kernel
  * of its own, us: rows 2 / 3 / 4 / 5 / 6 at the best of 2 to 4 blocks per SM
  * 98 / 94 / 91 / 90 / 92; in the program 4 rows at 2 blocks per SM lead (104
@@ -381,7 +382,6 @@ struct jacobi_fix_body {
 };
 
 #define JACOBI_SAMPLE 32768
-#define JACOBI_TRIES 3       /* FP64 sweeps after which a grid that few values keep from a window goes over */
 /* a sample of the grid's values.  elow = 0: their largest high word, in red->out how many no window can hold
  * (negative, infinite, NaN or above the highest) and, 2^16 each, how many are zero; else in red->out how many lie
  * outside the window that starts at elow */
@@ -406,14 +406,14 @@ static __device__ int jacobi_sample(const double *u, uint32_t cells, uint32_t el
 /* the lowest binade (biased exponent) of the fixed-point window that suits the grid u, 0 if none does: less
  * than one value in 4096 may lie outside it (each costs up to six points the FP64 path).  +0 lies in every
  * window; a sample of nothing else takes the one that ends at 2, and the first sweep sees what there is.
- * *fp64: the second kernel is the faster one for the grid: many values lie outside (of values uniform from 0 up to
- * one in 256 does, and none after a sweep), or `tries` sweeps have found no window; a grid with many zeros gains
- * nothing there. */
-static __device__ uint32_t jacobi_window(const double *u, uint32_t cells, int tries, bool *fp64, int *rc)
+ * *fp64: the second kernel is the faster one for the grid, because the values outside have not halved since the
+ * last sample (*outside; values that are spread at random fall into a window within a few sweeps, smooth or signed
+ * ones do not); a grid with many zeros gains nothing there. */
+static __device__ uint32_t jacobi_window(const double *u, uint32_t cells, uint32_t *outside, bool *fp64, int *rc)
 {
     jacobi_red red{0ull, 0, 0u};
     *rc = jacobi_sample(u, cells, 0u, &red);
-    const uint32_t top = (uint32_t)red.hi >> 20, zeros = red.out >> 16;
+    const uint32_t top = (uint32_t)red.hi >> 20, zeros = red.out >> 16, before = *outside;
     uint32_t bad = red.out & 0xffffu;
     *fp64 = false;
     if (!*rc && zeros == JACOBI_SAMPLE && bad == 0u)
@@ -424,7 +424,8 @@ static __device__ uint32_t jacobi_window(const double *u, uint32_t cells, int tr
         if (!*rc && bad <= JACOBI_SAMPLE / 4096)
             return top - 8u;
     }
-    *fp64 = zeros <= JACOBI_SAMPLE / 8 && (bad > JACOBI_SAMPLE / 128 || tries >= JACOBI_TRIES);
+    *outside = bad;
+    *fp64 = zeros <= JACOBI_SAMPLE / 8 && 2u * bad > before;
     return 0u;
 }
 
@@ -467,7 +468,7 @@ static __device__ jacobi_cut jacobi_make_cut(uint32_t nn, uint32_t warps)
  * integer add at 4 blocks per SM, 217 at 2).  The first kernel has the
  * fixed-point sweep, and FP64 sweeps for small grids, for the time between two
  * samples and for grids with many zeros.  The second one has the sweeps that
- * the options ask for, and takes over the grids that no window suits.
+ * the options ask for, and takes over the grids that no window will suit.
  */
 /* The fixed sweep is part of the worker loop: behind the trampoline pointer it took 111 us. */
 using jacobi_hot = gfd::hot_reduce<jacobi_red, GF_RED_MAX, jacobi_fix_body>;
@@ -484,14 +485,14 @@ GF_MAIN_HOT(jacobi, 2, jacobi_hot)(int argc, char **argv)
     const gf_udiv32 dt = gf_udiv32::make(cut.tiles);
     uint32_t elow = 0u;                            /* window of the fixed-point sweeps, 0: not known */
     int ask = 0, pause = 0;                        /* sweeps until the grid is sampled for a window (again) */
-    int tries = 0;                                 /* sweeps without a window */
+    uint32_t outside = 2u * JACOBI_SAMPLE;         /* sampled values outside the window, at the last failed sample */
     for (int s = 1; s <= job.sweeps; s++) {
         const double *u = owned ? owned : job.u0;
         double res = 0.0;
         int rc = 0;
         if (cells >= JACOBI_FIX_CELLS && !elow && ask-- == 0) {
             bool fp64;
-            elow = jacobi_window(u, cells, tries, &fp64, &rc);
+            elow = jacobi_window(u, cells, &outside, &fp64, &rc);
             ask = pause;
             pause = min(2 * pause + 1, 15);
             if (rc)
@@ -521,7 +522,6 @@ GF_MAIN_HOT(jacobi, 2, jacobi_hot)(int argc, char **argv)
         } else {
             rc = cells >= JACOBI_FIX_CELLS ? jacobi_sweep_ahead(u, un, nn, dn, dsk, &res)
                                            : jacobi_sweep<0>(u, un, nn, dn, cells, &res);
-            tries++;
         }
         if (rc)
             return 10;
