@@ -37,9 +37,9 @@ PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FP64_OPS_PER_POINT = 7
 # DRAM bytes (read + write) of one full launch (100 sweeps and the final
 # fwrite), from an ncu capture of the current program kernel on this
-# workload: dram__bytes_read.sum 14.392234 GB + dram__bytes_write.sum
-# 13.653888 GB.
-TRAFFIC_PER_LAUNCH = 14_392_233_728 + 13_653_888_256
+# workload: dram__bytes_read.sum 14.397905 GB + dram__bytes_write.sum
+# 13.663535 GB.
+TRAFFIC_PER_LAUNCH = 14_397_905_152 + 13_663_534_848
 
 
 def fp64_pipe_ops_per_point(int_adds):
@@ -426,7 +426,8 @@ def main():
                                  "sweeps_only": round(loop_bytes(N, 1) / sweep_s / 1e9, 1)}},
             "e2e": None if e2e is None else {"value": round(e2e, 2), "unit": "GB/s", "h2d_bytes_per_step": N ** 3 * 8,
                     "d2h_bytes_per_step": N ** 3 * 8 + 100 * 24, "steps": e2e_steps, "warmup": 1},
-            "gpu_launches": args.steps,
+            # a program: the reset kernel and its kernels (two where it may change over to the second)
+            "gpu_launches": args.steps * (3 if fixed else 2),
             "cpu_baseline": cpu,
             "cpu_openmp": cpu_omp,
             "clocks": clk.summary(),

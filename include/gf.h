@@ -367,7 +367,9 @@ GF_API int gf_alloc_e1(gf_ctx *ctx, int kind, uint32_t teams, uint32_t threads, 
 GF_API int gf_fp64_add_rate(uint32_t blocks, int64_t iters, void *stream, float *ms, double *adds);
 
 /* Number of SMs and resident blocks per SM that a program's grid uses at
- * `block` threads (for sizing, tests and roofline accounting). */
+ * `block` threads (for sizing, tests and roofline accounting): the first
+ * kernel's, where a program has two; a launch with a larger grid takes the
+ * second one if that has room for it. */
 GF_API int gf_grid_info(gf_ctx *ctx, gf_program prog, uint32_t *sms, uint32_t *blocks_per_sm);
 
 /* ------------------------------------------------------------------ allocation-free reduction */
