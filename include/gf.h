@@ -126,7 +126,9 @@ typedef struct gf_stats {
     uint64_t regions;             /* parallel regions run                                   */
     uint64_t region_ns;           /* device time inside regions (publish -> all blocks done) */
     uint64_t heap_alloc, heap_free, heap_fail, heap_bad_free;
-    uint64_t heap_live_bytes, heap_high_water;
+    uint64_t heap_live_bytes;
+    uint64_t heap_high_water;     /* most bytes live at once (a request above 64 KiB that fails
+                                     can show in another's reading)                         */
     uint64_t main_ns;             /* device time from main() entry to return               */
     uint64_t host_slots;          /* slots the host served (cumulative)                    */
     uint64_t host_records;        /* lane records the host served (cumulative)             */

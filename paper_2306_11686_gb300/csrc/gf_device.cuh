@@ -199,7 +199,7 @@ struct backoff {
  * thousands of groups waiting for a slot or a reply for hundreds of
  * microseconds; polling every 512 ns each, they crowd the host server's own
  * accesses to the ring off the link (2^16 x 4 printf with 8 and 16 server
- * threads, medians on three boxes: 3.5 to 3.9 and 3.0 to 3.4 ms so, 2.4 and 1.6
+ * threads, medians on three machines: 3.5 to 3.9 and 3.0 to 3.4 ms so, 2.4 and 1.6
  * now; sleeps of at most 8 us 3.5 and 3.2). */
 struct link_backoff {
     uint64_t t0, limit;

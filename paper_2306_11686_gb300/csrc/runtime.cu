@@ -754,7 +754,7 @@ extern "C" GF_API int gf_launch_q(gf_ctx *c, gf_program prog, int argc, const ch
     uint32_t per_sm = 0, per_sm2 = 0;
     int rc = resident(pe.occ, &per_sm);
     if (rc == GF_OK && pe2.pick)
-        rc = resident(pe2.occ, &per_sm2);
+        rc = resident(pe2.occ, &per_sm2);    /* which also loads it: a first launch behind a running program would wait for it */
     if (rc)
         return rc;
     const uint32_t sms = (uint32_t)c->nsm;
@@ -951,7 +951,7 @@ static int inst_start(gf_ctx *c, Instance *in, cudaStream_t stream, uint32_t gri
     a.ext = (uint64_t *)in->d_ext;
     a.ext0 = (uint64_t)in->npages << 32;
     /* Where programs run side by side, the heap's free stacks (0.85 MB) by a memset: cleared by the kernel, 16
-     * programs served at once took 59.6 ms for 57.0 (alternating runs on one box).  A memset of this size in front
+     * programs served at once took 59.6 ms for 57.0 (alternating runs on one machine).  A memset of this size in front
      * of the kernel or behind it is what it takes, a small one does not do; the programs' blocks land on the same
      * SMs either way, and why they then run faster is not known.  A context for one program saves the 5 us. */
     if (c->cfg.max_programs > 1) {
